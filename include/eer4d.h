@@ -128,8 +128,9 @@ int eer4d_plan_info(const eer4d_plan* plan, eer4d_info* h_info);
 
 /* Bytes the caller allocates: counts (the accumulation workspace of
  * ssb_accumulate), G (the resident spectrum) and scratch (the largest need of
- * com_dpc, ssb_reconstruct with n_cand candidates, ssb_grad and
- * ssb_variance_grad). */
+ * com_dpc, virtual_detectors, ssb_reconstruct with n_cand candidates, ssb_grad
+ * and ssb_variance_grad).  Scratch for n_cand serves every call with fewer
+ * candidates too (it never shrinks as n_cand grows). */
 int eer4d_workspace_bytes(const eer4d_plan* plan, int n_cand, size_t* counts_bytes,
                           size_t* G_bytes, size_t* scratch_bytes);
 
