@@ -334,7 +334,8 @@ int ssb_g_slices(const eer4d_plan* plan, const void* d_G, const int32_t* h_bins,
  * (and scan rotation) of dataset i.  Outputs: h_phase[i] (host array of device
  * pointers, the array or any entry NULL to skip) float [scan_ny_i][scan_nx_i];
  * d_var double [n_sets] (nullable).  d_scratch needs the bytes
- * eer4d_batched_scratch_bytes returns.  EINVAL when n_sets is out of range, a
+ * eer4d_batched_scratch_bytes returns; scratch for some datasets also serves a
+ * call with any of them.  EINVAL when n_sets is out of range, a
  * pointer is NULL or the detector geometries differ.  Stage events, if any,
  * are those of h_plans[0]. */
 #define EER4D_MAX_SETS 32

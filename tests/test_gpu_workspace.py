@@ -81,3 +81,33 @@ def test_fewer_candidates_than_sized_for(P, scan, sized):
         assert torch.equal(rec.reconstruct(cands[:n])[0][0], one[0])
         assert P.refocus.sweep(rec, cands[:n]).shape == (n,)
     assert rec.check() == 0
+
+
+def test_batched_scratch_serves_any_of_its_datasets(P):
+    """Sizes over nested lists (uneven sides, both norms, every order), then 16
+    scans of 256x256 whose scratch is given to seven and to one of them."""
+    sides = [(256, 256), (32, 32), (512, 512), (64, 96), (2, 4), (300, 100), (1024, 64), (256, 256)]
+    plans = [P.Plan(_geometry(*s), norm=int(i == 3)) for i, s in enumerate(sides)] * 2
+    for drop in range(len(plans)):
+        size = [P.batched_scratch_bytes(plans[drop:drop + k]) for k in range(1, len(plans) - drop + 1)]
+        assert all(a <= b for a, b in zip(size, size[1:])), drop
+        rest = plans[:drop] + plans[drop + 1:]
+        assert P.batched_scratch_bytes(rest) <= P.batched_scratch_bytes(plans), drop
+        assert P.batched_scratch_bytes(rest[::-1]) == P.batched_scratch_bytes(rest)
+
+    w = synth.workload(2, scan_ny=256, scan_nx=256, e_per_frame=5.0)
+    d = synth.generate(w, "cuda")
+    rec = P.Reconstructor(synth.geometry(w))
+    rec.load(d.idx, d.off)
+    recs = [rec] * 16
+    need = P.batched_scratch_bytes([r.plan for r in recs])
+    ab = torch.zeros(16, 5, dtype=torch.float64, device="cuda")
+    ab[:, 0] = torch.linspace(-100.0, 100.0, 16)
+    scratch, guard = _guarded(need)
+    for n in (16, 8, 7, 1):
+        assert P.batched_scratch_bytes([r.plan for r in recs[:n]]) <= need
+        ph, _ = P.reconstruct_batched(recs[:n], ab[:n], scratch=scratch)
+        assert bool((guard == 0xA5).all()), n
+        for i in {0, n - 1}:
+            assert torch.equal(ph[i], rec.reconstruct(ab[i])[0][0]), (n, i)
+    assert rec.check() == 0
