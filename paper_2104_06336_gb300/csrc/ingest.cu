@@ -250,11 +250,13 @@ __global__ void __launch_bounds__(kComThreads) k_com_from_sums(const long long* 
 // shared tile and writes counts[p][f] as fp16.  No global atomics; every (p, f)
 // of the chunk is written exactly once, zeros included.
 //
-// Counters.  A tile none of whose frames has more than 255 events (every
-// detector dose) counts in bytes, four frames per word; another one counts the
-// chunk's pixels in two or three passes of 16-bit counters in the same shared
-// memory.  Rows are padded by one word so the pixels of a frame fall in
-// different banks.
+// Counters.  A tile none of whose frames has more than 255 events counts in
+// bytes, four frames per word; another one counts half its frames at a time, in
+// 16-bit counters in the same words, 256 events of a frame in flight (the
+// chunk's pixels in two or three passes, each over all events again and 64 in
+// flight, before: whole accumulation of 512 x 512 frames, 553 pixels, of 300
+// events each 900 -> 653 us, of 1200 2422 -> 1221).  Rows are padded by one word
+// so the pixels of a frame fall in different banks.
 //
 // Pixel of an event.  The kept pixels of a detector row are one interval of
 // raw x (a row of a disk, or of a shard of it), so the table is one entry per
@@ -278,7 +280,7 @@ template <bool SUMS>
 __global__ void __launch_bounds__(kThreads, 4) k_scatter(
     const uint32_t* __restrict__ idx, uint64_t n_idx, const uint64_t* __restrict__ off,
     uint64_t first, uint64_t nfr, uint32_t WH, uint32_t H, DivMod dw, uint32_t bin_m,
-    uint32_t bin_one, const uint2* __restrict__ rows, int rows_smem, int P_pad, int TF, int PC, int PC16, DivMod nch,
+    uint32_t bin_one, const uint2* __restrict__ rows, int rows_smem, int P_pad, int TF, int PC, DivMod nch,
     uint32_t ntiles, int wide, uint64_t NR, __half* counts, long long* sums,
     unsigned long long* totals, uint64_t F, uint32_t* st) {
   pdl_begin();
@@ -361,14 +363,15 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter(
       }
     }
   };
-  // counts the events of frames jg, jg + nw, .. into the tile of bytes (or 16-bit
-  // words) of pixels [p0, p0 + pc): their first 64 are in v, the rest are loaded
-  // here; once: their sums and drops too (a frame is counted in several passes)
-  auto count = [&](auto bytes, int b, int jg, int j1, const uint32_t (&v)[8], int p0, int pc,
+  // counts the events of frames jg, jg + nw, .. below j1 into the tile of bytes (or
+  // 16-bit counters from frame jb on) of pixels [p0, p0 + pc): their first 64 are
+  // in v, the rest are loaded here, 64 (256) at a time; once: their sums and drops too
+  // (a frame is counted for every chunk of pixels)
+  const int TP = TF / 4 + 1;
+  auto count = [&](auto bytes, int b, int jg, int jb, int j1, const uint32_t (&v)[8], int p0, int pc,
                    uint64_t tf0, bool once) {
     constexpr bool B = decltype(bytes)::value;
     constexpr int SH = B ? 2 : 1;
-    const int TP = (TF >> SH) + 1;
     const uint32_t inc = 1u << ((32 >> SH) * (jg & ((1 << SH) - 1)));
     [[maybe_unused]] uint32_t my_x = 0u, my_y = 0u, my_n = 0u;  // lane f: sums of frame f
 #pragma unroll
@@ -376,13 +379,14 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter(
       const int j = jg + f * nw;
       const uint32_t n = j < j1 ? s_n[b][j] : 0u;
       // 32-bit sums: at most 65535 events of x, y < 32768; of at most 255 events
-      // the number rides in the top byte of x's
+      // the number rides in the top byte of x's, of more sn counts those dropped
       [[maybe_unused]] uint32_t sx = 0u, sy = 0u, sn = 0u;
-      uint32_t* col = tile + (j >> SH);
+      uint32_t* col = tile + ((j - jb) >> SH);
       auto one = [&](uint32_t e, bool has) {
         if (!has) return;
         if (e >= WH) {
           drop += once;
+          if (SUMS && !B) ++sn;
           return;
         }
         uint32_t x, y;
@@ -390,29 +394,33 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter(
         if constexpr (SUMS) {
           sx += B ? x + (1u << 24) : x;
           sy += y;
-          if (!B) ++sn;
         }
         const uint2 r = rows_smem ? srow[y] : __ldg(rows + y);
         const uint32_t t = x - r.x;  // raw pixels from the row's first kept one
         const int pp = (int)((r.y >> 16) + __umulhi(t, bin_m) + t * bin_one) - p0;
         if (t < (r.y & 0xffffu) && (unsigned)pp < (unsigned)pc &&
-            EER4D_IN_RANGE(pp * TP + (j >> SH), words, st))
+            EER4D_IN_RANGE(pp * TP + ((j - jb) >> SH), words, st))
           atomicAdd(col + pp * TP, inc);
       };
       one(v[2 * f], lane < n);
       one(v[2 * f + 1], lane + 32 < n);
-      for (uint32_t k = 64; k < n; k += 64) {
+      constexpr int NL = B ? 2 : 8;  // loads of a lane in flight
+      for (uint32_t k = 64; k < n; k += 32 * NL) {
         const uint32_t* q = idx + s_lo[b][j] + k + lane;
-        const bool h0 = k + lane < n, h1 = k + lane + 32 < n;
-        const uint32_t e0 = h0 ? __ldg(q) : 0u, e1 = h1 ? __ldg(q + 32) : 0u;
-        one(e0, h0);
-        one(e1, h1);
+        uint32_t e[NL];
+#pragma unroll
+        for (int i = 0; i < NL; ++i) e[i] = k + 32 * i + lane < n ? __ldg(q + 32 * i) : 0u;
+#pragma unroll
+        for (int i = 0; i < NL; ++i) {
+          if (!B && k + 32 * i >= n) break;  // the same on every lane
+          one(e[i], k + 32 * i + lane < n);
+        }
       }
       if constexpr (SUMS) {
         if (once) {
           const uint32_t rx = __reduce_add_sync(0xffffffffu, sx);
           const uint32_t ry = __reduce_add_sync(0xffffffffu, sy);
-          const uint32_t rn = B ? rx >> 24 : __reduce_add_sync(0xffffffffu, sn);
+          const uint32_t rn = B ? rx >> 24 : n - __reduce_add_sync(0xffffffffu, sn);
           if (lane == f) my_x = B ? rx & 0xffffffu : rx, my_y = ry, my_n = rn;
         }
       }
@@ -439,7 +447,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter(
   };
   // frames [j, j + 4) of pixel p (fp16 pairs) -> counts, those in [j0, j1)
   auto put4 = [&](int p, uint64_t tf0, int j, int j0, int j1, uint32_t a, uint32_t b) {
-    if (!EER4D_IN_RANGE((long long)p * (long long)NR + (long long)(tf0 + j) + 3,
+    if (j + 3 < j0 || j >= j1) return;
+    if (!EER4D_IN_RANGE((long long)p * (long long)NR + (long long)tf0 + (j + 4 <= j1 ? j + 3 : j1 - 1),
                         (long long)P_pad * (long long)NR, st))
       return;
     __half* dst = counts + (size_t)p * NR + tf0 + j;
@@ -490,11 +499,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter(
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = pre[i];
         if (jg + 4 * nw < j1) fetch(b, jg + 4 * nw, j1, pre);
-        count(std::true_type{}, b, jg, j1, v, p0, pc, tf0, p0 == 0);
+        count(std::true_type{}, b, jg, 0, j1, v, p0, pc, tf0, p0 == 0);
       }
       __syncthreads();
       prefetch_next();
-      const int TW = TF / 4, TP = TW + 1;
+      const int TW = TF / 4;
       if (wide && j0 == 0 && j1 == TF) {
         // a thread stays at eight frames of a row and steps down the rows
         const int qs = __ffs(TW / 2) - 1, step = kThreads >> qs;
@@ -525,23 +534,29 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter(
         }
       }
     } else {
-      const int TW = TF / 2, TP = TW + 1;
-      const int qs = __ffs(TW / 2) - 1;
-      for (int c0 = 0; c0 < pc; c0 += PC16) {
-        const int cn = pc - c0 < PC16 ? pc - c0 : PC16;
-        const bool once = p0 + c0 == 0;
-        for (int jg = j0 + warp; jg < j1; jg += 4 * nw) {
+      const int TH = TF / 2;                  // frames of a half: TF / 4 words of two
+      const int step = TF >= 8 ? 2 : 1;       // words stored at a time
+      const int qs = __ffs(TF / 4 / step) - 1;
+      for (int jb = 0; jb < TF; jb += TH) {
+        const int ja = jb > j0 ? jb : j0, je = jb + TH < j1 ? jb + TH : j1;
+        if (ja >= je) continue;  // uniform
+        // pre holds the first frames from ja on: of the task, or of its second half
+        for (int jg = ja + warp; jg < je; jg += 4 * nw) {
           uint32_t v[8];
-          fetch(b, jg, j1, v);
-          count(std::false_type{}, b, jg, j1, v, p0 + c0, cn, tf0, once);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] = pre[i];
+          if (jg + 4 * nw < je) fetch(b, jg + 4 * nw, je, pre);
+          count(std::false_type{}, b, jg, jb, je, v, p0, pc, tf0, p0 == 0);
         }
         __syncthreads();
-        if (c0 + PC16 >= pc) prefetch_next();
-        for (int i = threadIdx.x; i < cn << qs; i += kThreads) {
-          const int p = i >> qs, w = i & (TW / 2 - 1);
-          uint32_t* c = tile + p * TP + 2 * w;
-          const uint32_t w0 = c[0], w1 = c[1];
-          c[0] = c[1] = 0u;
+        if (je < j1) fetch(b, je + warp, j1, pre);
+        else prefetch_next();
+        for (int i = threadIdx.x; i < pc << qs; i += kThreads) {
+          const int p = i >> qs, w = (i & ((1 << qs) - 1)) * step;
+          uint32_t* c = tile + p * TP + w;
+          const uint32_t w0 = c[0], w1 = step == 2 ? c[1] : 0u;
+          c[0] = 0u;
+          if (step == 2) c[1] = 0u;
           uint32_t h01, h23;
           if (mx < 1024u) {
             h01 = to_half2(w0 | 0x64006400u);
@@ -554,9 +569,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter(
             h01 = *reinterpret_cast<const uint32_t*>(&a);
             h23 = *reinterpret_cast<const uint32_t*>(&d);
           }
-          put4(p0 + c0 + p, tf0, 4 * w, j0, j1, h01, h23);
+          put4(p0 + p, tf0, jb + 2 * w, ja, je, h01, h23);
         }
-        if (c0 + PC16 < pc) __syncthreads();
+        if (je < j1) __syncthreads();
       }
     }
     __syncthreads();
@@ -665,7 +680,6 @@ cudaError_t launch_scatter(const eer4d_plan* p, const uint32_t* idx, uint64_t n_
   const int NCH = (p->P_pad + PC - 1) / PC;
   const uint32_t W = p->g.det_w, H = p->g.det_h;
   const size_t words = ((size_t)PC * (TF / 4 + 1) + 3) / 4 * 4;
-  const int PC16 = (int)(words / (TF / 2 + 1));  // pixels of a pass of 16-bit counters
   // row table in shared memory unless the detector is very tall
   const int rows_smem = H <= kScatterRowsSmem;
   const size_t sm = 4 * (words + (rows_smem ? (2 * (size_t)H + 3) / 4 * 4 : 0));
@@ -692,7 +706,7 @@ cudaError_t launch_scatter(const eer4d_plan* p, const uint32_t* idx, uint64_t n_
   stage_begin(p, EER4D_STAGE_SCATTER, s);
   auto kl = with_sums ? k_scatter<true> : k_scatter<false>;
   launch(kl, (unsigned)grid, kThreads, sm, s, idx, n_idx, off, first, n, W * H, H, p->dw, p->bin_m,
-         p->bin_one, p->d_rowtab, rows_smem, p->P_pad, TF, PC, PC16, nch, (uint32_t)tiles, wide,
+         p->bin_one, p->d_rowtab, rows_smem, p->P_pad, TF, PC, nch, (uint32_t)tiles, wide,
          (uint64_t)p->cstride, counts, reinterpret_cast<long long*>(sums),
          reinterpret_cast<unsigned long long*>(totals), (uint64_t)p->F, st);
   count_launches(1);
