@@ -122,13 +122,15 @@ void count_launches(int n);
 // library is up to 16 small kernels: whole path at 32 x 32 93 -> 79 us, 144
 // kernels of an iterative DPC 1.05 -> 0.78 ms.  Captured launches keep plain
 // edges, whose boundaries are cheaper in a graph (eight replayed refocus steps
-// 726 against 769 us).
+// 726 against 769 us).  launch_as(false, ..) keeps a launch behind the end of the
+// kernel before.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 template <typename... K, typename... A>
-cudaError_t launch(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+cudaError_t launch_as(bool overlap, void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                      A&&... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -139,9 +141,13 @@ cudaError_t launch(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaS
   cfg.stream = s;
   cfg.attrs = &at;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  const bool plain = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
-  cfg.numAttrs = plain ? 0 : 1;
+  if (overlap && cudaStreamIsCapturing(s, &cap) == cudaSuccess) overlap = cap == cudaStreamCaptureStatusNone;
+  cfg.numAttrs = overlap ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+}
+template <typename... K, typename... A>
+cudaError_t launch(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  return launch_as(true, kern, grid, block, smem, s, static_cast<A&&>(args)...);
 }
 // EER4D_OK for cudaSuccess; otherwise records the error text for
 // eer4d_last_error and returns EER4D_ECUDA.
