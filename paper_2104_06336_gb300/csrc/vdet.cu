@@ -33,7 +33,8 @@ __device__ __noinline__ int exact_ring(uint32_t x, uint32_t y, double cx, double
 // index a thread.  A pixel is decided in float32 unless it is within float32's
 // error of an edge, and the centre and edges are formed once a block (double
 // precision runs at two lanes a cycle: 576 x 576 pixels took 16 us in it, a
-// thread each; now 10).
+// thread each; now 10).  The edges are searched by halving: one after another, 64
+// rings of 256 x 256 frames of 20 events took 93 us, 12 rings 29; now 56 and 21.
 constexpr int kTableThreads = 256;
 __global__ void __launch_bounds__(kTableThreads)
     k_ring_table(uint32_t WH, DivMod dw, const long long* __restrict__ totals, double cx_h,
@@ -78,8 +79,13 @@ __global__ void __launch_bounds__(kTableThreads)
     for (int k = 0; k < 8; ++k) {
       const float dx = (float)((int)x - ix) - gx, dy = (float)((int)y - iy) - gy;
       const float r2 = fmaf(dx, dx, __fmul_rn(dy, dy));
-      int c = 0;  // edges below the pixel
-      while (c <= R.n && s_hi[c] < r2) ++c;
+      int c = 0;  // edges below the pixel: s_hi ascends
+      for (int n = R.n + 1; n > 0;) {
+        const int h = n >> 1;
+        const bool up = s_hi[c + h] < r2;
+        c = up ? c + h + 1 : c;
+        n = up ? n - h - 1 : h;
+      }
       const bool sure = near && (c > R.n || r2 < s_lo[c]);
       const int ring = sure ? (c > R.n ? -1 : c - 1) : exact_ring(x, y, cx, cy, R);
       pack[k >> 2] |= (uint32_t)(ring & 255) << (8 * (k & 3));

@@ -132,3 +132,26 @@ def test_ring_counts_units(P, scan):
     ref = orc.virtual_detector_counts(idx.view(np.uint32), off, g["det_w"], g["det_h"], radii, *c)
     np.testing.assert_array_equal(got.cpu().numpy().reshape(len(radii) - 1, F), ref)
     assert rec.check() == 0
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 63, 64])
+def test_ring_search(P, n):
+    """The edges below a pixel, for odd and even numbers of them: equal edges
+    (empty rings), the first at 0 and above it, the last past the detector and
+    at infinity, edges on whole squared radii and between."""
+    rng = np.random.default_rng(n)
+    g = synth.geometry(synth.workload(5, scan_ny=10, scan_nx=10))
+    F = 100
+    rec = P.Reconstructor(g, alloc_counts=False)
+    idx, off = scan_events(g, F, rng)
+    ti, to = torch.from_numpy(idx).cuda(), torch.from_numpy(off).cuda()
+    for last, first in ((250.0, 0.0), (5000.0, 3.5), (float("inf"), 0.0)):
+        radii = np.sort(rng.uniform(0.0, 300.0, n + 1))
+        radii[::3] = np.round(radii[::3])
+        radii[1::4] = radii[:-1:4][:radii[1::4].size]
+        radii = np.sort(radii)
+        radii[0], radii[-1] = min(first, radii[0]), max(last, radii[-1])
+        got = rec.virtual_detectors(ti, to, list(radii), use_totals=False, cx=287.0, cy=290.5)
+        ref = orc.virtual_detector_counts(idx.view(np.uint32), off, g["det_w"], g["det_h"], list(radii), 287.0, 290.5)
+        np.testing.assert_array_equal(got.cpu().numpy().reshape(n, F), ref)
+    assert rec.check() == 0
