@@ -63,8 +63,9 @@ __device__ __forceinline__ float2 split_b(float2 z, float2 zm) {
 // c*in_sc; its spectrum value k goes to k*out_skx + a*out_sa + c*out_sc.  A CTA
 // takes TA consecutive rows a0..a0+TA-1 (TA even, a power of two) at c =
 // blockIdx.y + c0 and transforms pairs z = row_2b + i row_2b+1.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_rows_r2c(const T* in, float2* out, const __grid_constant__ FftDesc d, int nA,
+// BIG: radices above 16 too; without them 64 registers a thread, four CTAs per SM.
+template <typename T, bool BIG>
+__global__ void __launch_bounds__(kThreads, BIG ? 1 : 4) k_rows_r2c(const T* in, float2* out, const __grid_constant__ FftDesc d, int nA,
                                                        int TA, int c0, long long in_sa,
                                                        long long in_sc, long long out_skx,
                                                        long long out_sa, long long out_sc, int a_fast,
@@ -83,7 +84,7 @@ __global__ void __launch_bounds__(kThreads) k_rows_r2c(const T* in, float2* out,
       Af[2 * ((al >> 1) * pitch + n) + (al & 1)] = a < nA ? to_f<T>(row[n]) : 0.f;
   }
   __syncthreads();
-  const float2* res = fft_sm + fft_smem<1>(d, nb, pitch);
+  const float2* res = fft_sm + fft_smem<1, FFT_SMEM, false, BIG>(d, nb, pitch);
   const int nk = N / 2 + 1, sh = __ffs(TA) - 1;
   const int tot2 = TA * nk;
   for (int w = tid; w < tot2; w += blockDim.x) {
@@ -326,8 +327,7 @@ __global__ void k_transpose(const float2* __restrict__ in, float2* __restrict__ 
   }
 }
 
-// transforms per CTA: at most `most`, both buffers within 64 KB (three CTAs
-// per SM), at least one
+// transforms per CTA: at most `most`, both buffers within 64 KB, at least one
 int fft_nb(const FftDesc& d, int most) {
   int nb = most;
   while (nb > 1 && (size_t)2 * nb * fft_pitch(d, nb) * sizeof(float2) > 64 * 1024) nb >>= 1;
@@ -348,6 +348,11 @@ cudaError_t cols(const FftDesc& d, const float2* in, float2* out, int dir, int n
   // call 719 -> 668 us, the 336 x 200 path 563 -> 556)
   int nb = fft_nb(d, 16);
   while (nb > 4 && (ncols + nb - 1) / nb * nbatch < 152) nb >>= 1;
+  // two columns rather than one while two CTAs fit an SM and there are CTAs enough
+  // (whole accumulation, 560 pixels: 2048 x 256 3.62 -> 2.86 ms, 3000 x 100 3.69 ->
+  // 2.60; at 4096, where one CTA would fit, 1.75 -> 2.20; an image of 2048 x 256,
+  // 129 columns, 187 -> 192 us)
+  if (nb == 1 && ncols / 2 * nbatch >= 152 && fft_bytes(d, 2) <= 110 * 1024) nb = 2;
   const int pitch = fft_pitch(d, nb);
   const size_t sm = fft_bytes(d, nb);
   auto kern = dir > 0 ? k_fft_cols<1> : k_fft_cols<-1>;
@@ -456,12 +461,16 @@ cudaError_t launch_stage1(const eer4d_plan* p, const __half* counts, float2* G, 
   const int nb = fft_nb(d, 8);
   const int TA = 2 * nb;
   const size_t sm = fft_bytes(d, nb);
-  cudaError_t e = set_smem(k_rows_r2c<__half>, sm);
+  // short rows are little work for a CTA between its barriers: four CTAs per SM
+  // where shared memory holds them (4096 x 64, 560 pixels, plain form 3.29 ->
+  // 2.51 ms); otherwise the registers (64 x 4096 1.07 ms, with 64 of them 1.18)
+  auto kern = fft_big(d) || sm > 56 * 1024 ? k_rows_r2c<__half, true> : k_rows_r2c<__half, false>;
+  cudaError_t e = set_smem(kern, sm);
   if (e != cudaSuccess) return e;
   const long long NR = p->cstride;
   dim3 grid((p->P_pad + TA - 1) / TA, y1 - y0);
   stage_begin(p, EER4D_STAGE_DFT_X, s);
-  launch(k_rows_r2c<__half>, grid, kThreads, sm, s, counts, G, d, p->P_pad, TA, y0, NR,
+  launch(kern, grid, kThreads, sm, s, counts, G, d, p->P_pad, TA, y0, NR,
          (long long)p->g.scan_nx, (long long)p->g.scan_ny * p->P_pad, 1, (long long)p->P_pad, 1,
          fft_pitch(d, nb));
   count_launches(1);
@@ -539,10 +548,11 @@ cudaError_t launch_r2c_image(const eer4d_plan* p, const float* g, float2* W, cud
   const FftDesc& d = p->fx;
   const int nb = fft_nb(d, 4), TA = 2 * nb;
   const size_t sm = fft_bytes(d, nb);
-  cudaError_t e = set_smem(k_rows_r2c<float>, sm);
+  auto kern = k_rows_r2c<float, true>;
+  cudaError_t e = set_smem(kern, sm);
   if (e != cudaSuccess) return e;
   dim3 grid((Ny + TA - 1) / TA, 1);
-  launch(k_rows_r2c<float>, grid, kThreads, sm, s, g, W, d, Ny, TA, 0, Nx, 0, 1, nkx, 0, 0,
+  launch(kern, grid, kThreads, sm, s, g, W, d, Ny, TA, 0, Nx, 0, 1, nkx, 0, 0,
          fft_pitch(d, nb));
   count_launches(1);
   e = cudaGetLastError();
