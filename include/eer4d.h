@@ -427,9 +427,10 @@ int eer4d_dft_split_factors(int n, int n_k, uint16_t* h_hi, uint16_t* h_lo);
 /* ---- launch-shape autotuner (not part of the method) --------------------------
  * Tile and grid shapes of the three main kernels.  Zero means the built-in
  * choice.  scatter_tf: frames per scatter tile (a power of two, 4..128);
- * *_ctas_per_sm: resident CTAs per SM of the persistent grids of the scatter,
- * the scan DFT of both axes and the trotter kernel (capped by occupancy).  ms: the
- * times (ms) the autotuner measured for its choices (scatter, DFT, trotter). */
+ * *_ctas_per_sm: resident CTAs per SM of the persistent grids of the scatter
+ * (3 and more: all that fit), the scan DFT of both axes and the trotter kernel
+ * (capped by occupancy; mixed-radix scan DFTs have no such grid).  ms: the times
+ * (ms) the autotuner measured for its choices (scatter, DFT, trotter). */
 typedef struct eer4d_tuning {
   int32_t scatter_tf;
   int32_t scatter_ctas_per_sm;
@@ -438,7 +439,7 @@ typedef struct eer4d_tuning {
   float   ms[3];
 } eer4d_tuning;
 /* Times the candidate shapes on the caller's data and keeps the fastest in the
- * plan: scatter (16..128 frames per tile x 1..3 CTAs/SM) over
+ * plan: scatter (16..128 frames per tile x 1, 2 or 3 CTAs/SM) over
  * the whole CSR (d_idx, d_off for all scan_ny*scan_nx frames), the scan
  * DFT of both axes (1..4 CTAs/SM; plans without it keep 0) and the trotter kernel with the
  * aberrations d_aberr (double[5]) (1..3 CTAs/SM).  d_work, d_G and d_scratch

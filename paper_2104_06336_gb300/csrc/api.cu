@@ -762,7 +762,7 @@ int eer4d_autotune(eer4d_plan* p, const uint32_t* d_idx, uint64_t n_idx, const u
   const eer4d_tuning keep = p->tune;
   eer4d_tuning best = keep;
   int rc = EER4D_OK;
-  // scatter: frames per tile 16..128 (pixels chunked to fit) x 1..3 CTAs per SM
+  // scatter: frames per tile 16..128 (pixels chunked to fit) x 1, 2 or all CTAs that fit an SM
   {
     float tbest = -1.f;
     for (int tf = 16; tf <= 128; tf *= 2) {

@@ -706,8 +706,12 @@ cudaError_t launch_scatter(const eer4d_plan* p, const uint32_t* idx, uint64_t n_
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, sm);
   if (occ < 1) return cudaErrorInvalidConfiguration;  // the tile does not fit shared memory
-  const int cps = p->tune.scatter_ctas_per_sm > 0 && p->tune.scatter_ctas_per_sm < occ
-                      ? p->tune.scatter_ctas_per_sm : occ;
+  // tuned values from kScatterAll on mean all the CTAs that fit (kept tunings were
+  // made when that was three at most): 1024 x 1024 frames of 50 events, 553 pixels,
+  // 341 us with three, 325 with the four that fit
+  constexpr int kScatterAll = 3;
+  const int most = p->tune.scatter_ctas_per_sm;
+  const int cps = most > 0 && most < kScatterAll && most < occ ? most : occ;
   uint64_t grid = (uint64_t)nsm * cps;
   if (grid > tiles) grid = tiles;
   stage_begin(p, EER4D_STAGE_SCATTER, s);
