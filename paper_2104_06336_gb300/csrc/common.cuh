@@ -94,6 +94,7 @@ struct eer4d_plan {
   uint32_t* d_tl_e;
   int4* d_tl_at;             // per warp task: first entry, entries of the two sets
   int* d_tl_order;           // warp tasks by decreasing list length (work-queue order)
+  int tl_n;                  // words of d_tl_bits and of d_tl_e
   float2* d_tw_y;            // [scan_ny] (+ [scan_ny] four-step layout, FftDesc)
   float2* d_tw_x;            // [scan_nx] (+ [scan_nx])
   float2* d_tw_y2;           // [2 scan_ny] (+ [2 scan_ny]; zero-padded DPC grid)

@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
       carry = __shfl_sync(0xffffffffu, v[3], 31);
     }
     const int k = c + 4 * lane;
+    if (!EER4D_IN_RANGE(lo - pad + (k + 4 <= m ? k + 3 : m - 1), n, st)) continue;
     if (VEC && k >= pad && k + 4 <= m) {
       *reinterpret_cast<uint4*>(dst + k) = make_uint4(v[0], v[1], v[2], v[3]);
     } else {

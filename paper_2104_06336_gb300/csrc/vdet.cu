@@ -167,8 +167,10 @@ __global__ void __launch_bounds__(kWarps * 32, 5)
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             int* c = cnt + (s + q) * pitch;
-            if (has[2 * q] && ring[2 * q] != 255) atomicAdd(c + ring[2 * q], 1);
-            if (has[2 * q + 1] && ring[2 * q + 1] != 255) atomicAdd(c + ring[2 * q + 1], 1);
+            if (has[2 * q] && ring[2 * q] != 255 && EER4D_IN_RANGE(ring[2 * q], n_rings, st))
+              atomicAdd(c + ring[2 * q], 1);
+            if (has[2 * q + 1] && ring[2 * q + 1] != 255 && EER4D_IN_RANGE(ring[2 * q + 1], n_rings, st))
+              atomicAdd(c + ring[2 * q + 1], 1);
           }
         }
       }

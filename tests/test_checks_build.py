@@ -90,3 +90,58 @@ def test_small_workloads_pass_every_bounds_check(checks_lib):
         assert rel[k]["status"] == 0
         for f in ("G", "counts", "sums", "ph", "var", "g", "ph_rot"):
             assert dbg[k][f] == rel[k][f], (k, f)
+
+
+_CHILD_EVENTS = r"""
+import json, sys
+import numpy as np, torch
+sys.path.insert(0, ROOT)
+import paper_2104_06336_gb300 as P
+import synth
+out = {}
+def total(t):
+    return float(t.double().abs().sum())
+rng = np.random.default_rng(5)
+for scan, norm, tf in (((34, 30), 0, 4), ((10, 10), 1, 128), ((48, 64), 0, 0)):
+    g = synth.geometry(synth.workload(5, scan_ny=scan[0], scan_nx=scan[1]))
+    F = scan[0] * scan[1]
+    n = rng.integers(0, 90, F)
+    n[::37] = 700  # 16-bit counters
+    off = torch.from_numpy(np.concatenate([[0], np.cumsum(n)])).cuda()
+    idx = torch.from_numpy(rng.integers(0, g["det_w"] * g["det_h"], int(n.sum())).astype(np.int32)).cuda()
+    rec = P.Reconstructor(g, norm=norm, n_cand=9)
+    if tf:
+        P.eer4d_set_tuning(rec.plan, dict(P.eer4d_get_tuning(rec.plan), scatter_tf=tf))
+    r = {}
+    for chunk in (None, F // 3 + 1):
+        rec.load(idx, off, chunk_frames=chunk)
+        r[f"counts{chunk}"], r[f"G{chunk}"] = total(rec.counts), total(rec.G)
+    runs = torch.from_numpy(rng.integers(0, 300, int(n.sum())).astype(np.int32)).cuda()
+    r["rle"] = total(P.eer_decode_rle(runs, off, status=rec.status))
+    r["rle1"] = total(P.eer_decode_rle(runs[1:], (off - 1).clamp(min=0), status=rec.status))
+    r["rings"] = total(rec.virtual_detectors(idx, off, [0.0, 40.0, 97.5, 200.0]))
+    ab = torch.zeros(9, 5, dtype=torch.float64)
+    ab[:, 0] = torch.linspace(-80.0, 80.0, 9)
+    for rot in (0.0, 0.4):
+        ab[:, 4] = rot
+        r[f"cand{rot}"] = total(rec.reconstruct(ab)[0])
+        r[f"counts{rot}"] = total(rec.trotter_counts(rot))
+        r[f"grad{rot}"] = rec.variance_grad(ab[1])[1].cpu().numpy().tolist()
+    sums, com, dpc = rec.com_dpc(idx, off)
+    r["dpc"] = total(rec.dpc_iterative(com, 3))
+    torch.cuda.synchronize()
+    r["status"] = P.status_code(rec.status)
+    out[f"{scan}{norm}{tf}"] = r
+print("RESULT" + json.dumps(out))
+"""
+
+
+@pytest.mark.gpu
+def test_event_and_list_paths_pass_every_bounds_check(checks_lib, monkeypatch):
+    """16-bit counters, frames per task of 4 and 128, streamed ranges, run-length
+    decoding on and off 16 bytes, ring counts, lists and set tests, both norms."""
+    from paper_2104_06336_gb300.buildlib import build
+    monkeypatch.setattr(sys.modules[__name__], "_CHILD", _CHILD_EVENTS)
+    rel, dbg = _run(build()), _run(checks_lib)
+    assert rel == dbg
+    assert all(r["status"] == 0 for r in rel.values()), rel
