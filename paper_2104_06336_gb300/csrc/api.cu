@@ -139,7 +139,6 @@ void free_plan(eer4d_plan* p) {
   cudaFree(p->d_rowtab);
   cudaFree(p->d_pix);
   cudaFree(p->d_bfp);
-  cudaFree(p->d_rows);
   cudaFree(p->d_tl_bits);
   cudaFree(p->d_tl_e);
   cudaFree(p->d_tl_at);
@@ -314,7 +313,6 @@ static int create_plan(const eer4d_geom* h_geom, int precision, int norm, int sh
   p->P_bf = P_bf;
   p->P_pad = (p->P + 15) / 16 * 16;
   p->n_rows = (int)rows.size();
-  p->list_max = (P_bf + 1) & ~1;
   pix.resize(p->P_pad, make_short2(0, 0));
   std::vector<int32_t> bfp;  // kept-pixel index of every bright-field pixel, row-major
   for (const int4& R : rows)
@@ -339,7 +337,6 @@ static int create_plan(const eer4d_geom* h_geom, int precision, int norm, int sh
   cudaError_t e;
   if ((e = upload(&p->d_rowtab, rowtab)) != cudaSuccess || (e = upload(&p->d_pix, pix)) != cudaSuccess ||
       (e = upload(&p->d_bfp, bfp)) != cudaSuccess ||
-      (e = upload(&p->d_rows, rows)) != cudaSuccess ||
       (e = make_fft((int)g.scan_ny, p->fy, &p->d_tw_y)) != cudaSuccess ||
       (e = make_fft((int)g.scan_nx, p->fx, &p->d_tw_x)) != cudaSuccess ||
       (e = make_fft(2 * (int)g.scan_ny, p->fy2, &p->d_tw_y2)) != cudaSuccess ||

@@ -10,6 +10,10 @@
 #define EER4D_MAX_STAGES 16
 #define EER4D_WARPS_TROTTER 4
 
+// SMs of the GPU this is written for: how finely small problems are cut.  Grids
+// that have to match the residency ask the device.
+constexpr int kSms = 152;
+
 // ---------------------------------------------------------------- complex ---
 __host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
@@ -18,10 +22,6 @@ __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 }
 __host__ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __host__ __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
-// multiply by -i (dir = +1) or +i (dir = -1)
-__device__ __forceinline__ float2 cmul_mi(float2 a, int dir) {
-  return dir > 0 ? make_float2(a.y, -a.x) : make_float2(-a.y, a.x);
-}
 
 // ------------------------------------------------------- integer division ---
 // Exact floor division of a uint32 by a runtime divisor d >= 1:
@@ -71,7 +71,7 @@ struct FftDesc {
 struct eer4d_plan {
   eer4d_geom g;
   int precision, norm;
-  int P, P_pad, P_bf, n_rows, nkx, list_max;
+  int P, P_pad, P_bf, n_rows, nkx;
   // pixel shard: this plan owns the kept pixels [p_begin, p_end) of the full
   // plan's numbering (shard of n_shards; 0 of 1 for an ordinary plan)
   int shard, n_shards, p_begin, p_end;
@@ -89,7 +89,6 @@ struct eer4d_plan {
   __half* d_dft_lo;
   unsigned char* d_tc4_tabs;  // four-step tensor-core DFT: split factor matrices (SPLIT_FP16, 1024 columns)
   float2* d_tc4_tw;           // and its twiddles W1024^(xl kl) / 2 [32][17]
-  int4* d_rows;              // [n_rows] (ky, bf kx lo, bf kx hi, p at bf lo)
   uint32_t* d_tl_bits;       // trotter membership lists at rotation 0 (d_tl_at NULL: none)
   uint32_t* d_tl_e;
   int4* d_tl_at;             // per warp task: first entry, entries of the two sets
@@ -182,26 +181,10 @@ __device__ __forceinline__ bool eer4d_in_range(long long i, long long n, uint32_
 #endif
 
 // ------------------------------------------------------------ warp helpers ---
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 __device__ __forceinline__ long long warp_sum_ll(long long v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-__device__ __forceinline__ int warp_excl_scan(int v, int& total) {
-  int lane = threadIdx.x & 31;
-  int x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  total = __shfl_sync(0xffffffffu, x, 31);
-  return x - v;
 }
 
 // signed frequency index of bin m of an N-point DFT (numpy fftfreq order)

@@ -176,6 +176,7 @@ __global__ void __launch_bounds__(R1 * CP, EER4D_DFT2_MINB * 128 / (R1 * CP))
                  const float2* __restrict__ twx4, const float2* __restrict__ twy4, Dft2Params q,
                  unsigned* ctl, uint32_t* st) {
   pdl_begin();
+  static_assert(R1 == 32 && R2 == 32, "s1_tile_w32");
   constexpr int NT = R1 * CP;
   constexpr int N = R1 * R2;  // = q.N
   constexpr int GP = 2 * CP;  // pixels per group, = q.gp

@@ -11,10 +11,13 @@
 namespace {
 
 constexpr int kThreads = 256;
-// k_gen_rows and k_rows_c2c: few transforms in small CTAs, eight per SM (seven
-// where registers hold a radix above 16), whose barriers wait for less.  (336 x 200
-// whole path 498 us, with eight 543, six 519; without radices above 16 586, and at
-// 256 threads and twice the transforms 621; 300 x 128 343 and 444.)
+// k_gen_rows and k_rows_c2c: few transforms in small CTAs, whose barriers wait for
+// less; registers for eight CTAs per SM (seven where they hold a radix above 16),
+// of which shared memory leaves eight with rows of 200 points, five with 336 and
+// four with 400.  (Scan DFT of 336 x 200 positions, 1248 pixels, 328 us; budgets of
+// six, eight and five CTAs 341, 373 and 396; 200 x 336 377, 402, 387, 451; without
+// radices above 16, 300 x 128 with eight 207, six 211, 90 x 66 72 and 78.  Longer
+// rows do not tell eight, seven and six apart: 800 x 600, 1000 x 1000.)
 constexpr int kDirectThreads = 128;
 constexpr int direct_blocks(bool big) { return big ? 7 : 8; }
 
@@ -347,12 +350,12 @@ cudaError_t cols(const FftDesc& d, const float2* in, float2* out, int dir, int n
   // a launch of a few CTAs lasts as long as one of them (16 uneven scans in one
   // call 719 -> 668 us, the 336 x 200 path 563 -> 556)
   int nb = fft_nb(d, 16);
-  while (nb > 4 && (ncols + nb - 1) / nb * nbatch < 152) nb >>= 1;
+  while (nb > 4 && (ncols + nb - 1) / nb * nbatch < kSms) nb >>= 1;
   // two columns rather than one while two CTAs fit an SM and there are CTAs enough
   // (whole accumulation, 560 pixels: 2048 x 256 3.62 -> 2.86 ms, 3000 x 100 3.69 ->
   // 2.60; at 4096, where one CTA would fit, 1.75 -> 2.20; an image of 2048 x 256,
   // 129 columns, 187 -> 192 us)
-  if (nb == 1 && ncols / 2 * nbatch >= 152 && fft_bytes(d, 2) <= 110 * 1024) nb = 2;
+  if (nb == 1 && ncols / 2 * nbatch >= kSms && fft_bytes(d, 2) <= 110 * 1024) nb = 2;
   const int pitch = fft_pitch(d, nb);
   const size_t sm = fft_bytes(d, nb);
   auto kern = dir > 0 ? k_fft_cols<1> : k_fft_cols<-1>;

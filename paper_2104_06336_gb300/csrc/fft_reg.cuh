@@ -231,24 +231,23 @@ __global__ void __launch_bounds__((R1 > R2 ? R1 : R2) * CB, 768 / ((R1 > R2 ? R1
 
 // Real rows (fp16 counts) -> half spectra, scan DFT along x of the G function.
 // Row (a, c) = (pixel, scan row y) starts at a*in_sa + c*in_sc; spectrum value
-// k goes to k*out_skx + (a - a_out0)*out_sa + c*out_sc.  The tile takes 2*CP
+// k goes to k*out_skx + a*out_sa + c*out_sc.  The tile takes 2*CP
 // consecutive pixels from a0 at scan row c and transforms them as CP complex
 // rows z = row_2b + i row_2b+1; A(k) = (Z(k) + conj Z(-k))/2,
 // B(k) = -i (Z(k) - conj Z(-k))/2.  Requires R1 >= R2 so pass 2 has exactly
 // one (k1, b) group per thread.  `sm` holds max(R1*CP*(R2+1), N*CP) float2.
-// FULL: the caller guarantees a0 + 2*CP <= nA (no bounds tests).
-template <int R1, int R2, int CP, bool STREAM, bool FULL = false>
+template <int R1, int R2, int CP>
 __device__ __forceinline__ void rowfft_r2c_tile(const __half* __restrict__ in, float2* out,
                                                 const float2* __restrict__ tw4, int nA, int a0,
-                                                int a_out0, int c, long long in_sa,
-                                                long long in_sc, long long out_skx,
-                                                long long out_sa, long long out_sc, float2* sm) {
+                                                int c, long long in_sa, long long in_sc,
+                                                long long out_skx, long long out_sa,
+                                                long long out_sc, float2* sm) {
   static_assert(R1 >= R2, "R1 >= R2");
   static_assert(R1 == reg_r1(R1 * R2), "twiddle layout of FftDesc::tw4");
   constexpr int N = R1 * R2;
   constexpr int NT = R1 * CP;
   constexpr int PITCH = R2 + 1;
-  const bool full = FULL || a0 + 2 * CP <= nA;  // every pixel row of the tile exists
+  const bool full = a0 + 2 * CP <= nA;  // every pixel row of the tile exists
   for (int g = threadIdx.x; g < R2 * CP; g += NT) {
     const int j2 = g % R2, b = g / R2;
     const int ra = a0 + 2 * b, rb = ra + 1;
@@ -258,12 +257,12 @@ __device__ __forceinline__ void rowfft_r2c_tile(const __half* __restrict__ in, f
     if (full) {
 #pragma unroll
       for (int j1 = 0; j1 < R1; ++j1)
-        v[j1] = make_float2(ld_h<STREAM>(pa + R2 * j1), ld_h<STREAM>(pb + R2 * j1));
+        v[j1] = make_float2(ld_h<false>(pa + R2 * j1), ld_h<false>(pb + R2 * j1));
     } else {
 #pragma unroll
       for (int j1 = 0; j1 < R1; ++j1) {
-        const float xa = ra < nA ? ld_h<STREAM>(pa + R2 * j1) : 0.f;
-        const float xb = rb < nA ? ld_h<STREAM>(pb + R2 * j1) : 0.f;
+        const float xa = ra < nA ? ld_h<false>(pa + R2 * j1) : 0.f;
+        const float xb = rb < nA ? ld_h<false>(pb + R2 * j1) : 0.f;
         v[j1] = make_float2(xa, xb);
       }
     }
@@ -288,22 +287,22 @@ __device__ __forceinline__ void rowfft_r2c_tile(const __half* __restrict__ in, f
   __syncthreads();
   // one thread per (k, pair b): both half spectra from Z(k) and Z(-k).  With
   // out_sa == 1 the pair's two values are adjacent and go out as one 16-byte
-  // store (callers keep out, out_skx, out_sc and a0 - a_out0 even).
+  // store (callers keep out, out_skx, out_sc and a0 even).
   constexpr int NK = N / 2 + 1;
   for (int w = threadIdx.x; w < NK * CP; w += NT) {
     const int b = w % CP, k = w / CP;
     const int a = a0 + 2 * b;
-    if (!FULL && a >= nA) continue;
+    if (a >= nA) continue;
     const float2 z = sm[k * CP + b];
     const float2 zm = sm[((N - k) & (N - 1)) * CP + b];
     const float2 A = make_float2(0.5f * (z.x + zm.x), 0.5f * (z.y - zm.y));
     const float2 B = make_float2(0.5f * (z.y + zm.y), -0.5f * (z.x - zm.x));
-    float2* o = out + k * out_skx + (a - a_out0) * out_sa + c * out_sc;
-    if (out_sa == 1 && (FULL || a + 1 < nA)) {
+    float2* o = out + k * out_skx + a * out_sa + c * out_sc;
+    if (out_sa == 1 && a + 1 < nA) {
       *reinterpret_cast<float4*>(o) = make_float4(A.x, A.y, B.x, B.y);
     } else {
       o[0] = A;
-      if (FULL || a + 1 < nA) o[out_sa] = B;
+      if (a + 1 < nA) o[out_sa] = B;
     }
   }
 }
@@ -316,6 +315,6 @@ __global__ void __launch_bounds__(R1 * CP, 768 / (R1 * CP))
                      long long out_sa, long long out_sc) {
   pdl_begin();
   extern __shared__ float2 sm[];
-  rowfft_r2c_tile<R1, R2, CP, false>(in, out, tw4, nA, blockIdx.x * 2 * CP, 0, c0 + blockIdx.y,
-                                     in_sa, in_sc, out_skx, out_sa, out_sc, sm);
+  rowfft_r2c_tile<R1, R2, CP>(in, out, tw4, nA, blockIdx.x * 2 * CP, c0 + blockIdx.y, in_sa, in_sc,
+                              out_skx, out_sa, out_sc, sm);
 }

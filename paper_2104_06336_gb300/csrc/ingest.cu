@@ -619,7 +619,7 @@ int scatter_tf_for(const eer4d_plan* p) {
     const int pc = scatter_pc(p->P_pad, tf);
     return (long long)(p->F / tf) * ((p->P_pad + pc - 1) / pc);
   };
-  while (tf > 16 && tasks() < 2 * 152)
+  while (tf > 16 && tasks() < 2 * kSms)
     tf /= 2;
   return tf;
 }
@@ -632,7 +632,7 @@ cudaError_t launch_validate(const eer4d_plan* p, const uint32_t* idx, uint64_t n
   // one full wave of 152 SMs, no partial second one (resident CTAs of 48 registers
   // a thread, 64 with the PACBED)
   auto kv = pacbed ? k_validate<true> : k_validate<false>;
-  const uint64_t wave = 152 * (pacbed ? 4 : 5);
+  const uint64_t wave = kSms * (pacbed ? 4 : 5);
   if (blocks > wave) blocks = wave;
   if (blocks == 0) blocks = 1;
   stage_begin(p, EER4D_STAGE_VALIDATE, s);

@@ -168,8 +168,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 cudaError_t launch_rle_decode(const uint32_t* runs, uint64_t n, const uint64_t* off,
                               uint64_t n_frames, uint32_t* idx, uint32_t* st, cudaStream_t s) {
   if (n_frames == 0) return cudaSuccess;
-  // frames of a warp: enough warps to fill the GPU first (152 SMs x 48)
-  const uint64_t want = n_frames / (152 * 48);
+  // frames of a warp: enough warps to fill the GPU first (48 per SM)
+  const uint64_t want = n_frames / (kSms * 48);
   const int per_warp = want < 1 ? 1 : want > 32 ? 32 : (int)want;
   const uint64_t blocks = (n_frames + (uint64_t)kWarpsPerBlock * per_warp - 1) / ((uint64_t)kWarpsPerBlock * per_warp);
   const uintptr_t pr = reinterpret_cast<uintptr_t>(runs), pi = reinterpret_cast<uintptr_t>(idx);

@@ -199,7 +199,7 @@ cudaError_t launch_virtual_detectors(const eer4d_plan* p, const uint32_t* idx, u
   for (int j = n_rings + 1; j <= EER4D_MAX_RINGS; ++j) R.r2[j] = 0.0;
   unsigned char* lut = static_cast<unsigned char*>(scratch);
   const uint32_t WH = p->g.det_w * p->g.det_h;
-  launch(k_ring_table, 152, kTableThreads, 0, s, WH, p->dw, reinterpret_cast<const long long*>(totals), cx,
+  launch(k_ring_table, kSms, kTableThreads, 0, s, WH, p->dw, reinterpret_cast<const long long*>(totals), cx,
          cy, R, lut);
   count_launches(1);
   if (n_frames == 0) return cudaGetLastError();
@@ -207,7 +207,7 @@ cudaError_t launch_virtual_detectors(const eer4d_plan* p, const uint32_t* idx, u
   // work, 32 (128-byte rows of counts) at most, the counts of a block within 28 KB.
   const size_t frame = sizeof(int) * (size_t)(n_rings | 1) * kWarps;
   int per_log2 = 2;
-  while (per_log2 < 5 && (n_frames >> (per_log2 + 1)) >= 152 * 32 && frame << (per_log2 + 1) <= 28 * 1024) ++per_log2;
+  while (per_log2 < 5 && (n_frames >> (per_log2 + 1)) >= kSms * 32 && frame << (per_log2 + 1) <= 28 * 1024) ++per_log2;
   const size_t sm = frame << per_log2;
   const uint64_t span = (uint64_t)kWarps << per_log2;
   const uint64_t blocks = (n_frames + span - 1) / span;
