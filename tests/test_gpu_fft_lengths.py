@@ -55,5 +55,5 @@ def test_lengths_match_oracle(P, scan):
     g = rec.grad(torch.tensor(th, dtype=torch.float64), torch.from_numpy(u).cuda()).cpu().numpy()
     gr = orc.ssb_grad(G, geom, th, u.astype(np.float64))
     scales = np.array([100.0, 50.0, 50.0, 1.0e4, 0.1])
-    assert np.all(np.abs(g - gr) * scales <= 2e-4 * np.max(np.abs(gr) * scales))
+    assert np.all(np.abs(g - gr) * scales <= 1e-4 * np.max(np.abs(gr) * scales))
     assert rec.check() == 0
