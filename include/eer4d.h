@@ -67,8 +67,8 @@ extern "C" {
                                    y at the end) through a full-size intermediate; the
                                    same arithmetic as EER4D_FP32_FFT */
 #define EER4D_FP32_STOCKHAM 3   /* the plain form: FP32 shared-memory Stockham FFT
-                                   (radix 8/4/2 and odd primes) for both axes, two
-                                   launches plus a transpose */
+                                   (radices 2 to 24, larger primes by direct sums) for
+                                   both axes, two launches plus a transpose */
 #define EER4D_NORM_NONE  0  /* Eq. 3 as printed: S(K) = sum over K(K) */
 #define EER4D_NORM_AREA  1  /* S(K) / |K(K)| (0 when the set is empty) */
 
@@ -223,13 +223,17 @@ int dpc_iterative(const eer4d_plan* plan, const float* d_com, double lam1, doubl
  * the start of the workspace d_counts (fp16 [P_pad][scan_ny*scan_nx], exact
  * integers up to 2048; eer4d_workspace_bytes gives the workspace size).  The
  * rest of the workspace (from the next 256-byte boundary) holds the
- * intermediate of the scan DFT:
- *  - FP32_FFT plans whose scan sides are both 128, 256, 512 or 1024: nothing
- *    until is_last; then both axes, at 1024 x 1024 in one persistent launch
- *    through a ring of four pixel-group slabs (the two in use kept in L2) and
- *    its task counters, otherwise in two launches in place on d_G;
- *  - otherwise: the DFT along x of every scan row completed by this chunk,
- *    complex64 [scan_nx/2+1][scan_ny][P_pad]; with is_last the DFT along y.
+ * intermediate of the scan DFT, if it needs one:
+ *  - FP32_FFT plans of 1024 x 1024 scans: nothing until is_last; then both axes
+ *    in one persistent launch through a ring of four pixel-group slabs (the two
+ *    in use kept in L2) and its task counters;
+ *  - FP32_FFT plans whose sides are both 128, 256, 512 or 1024 otherwise, or both
+ *    at most 1024 and not both powers of two from 16 up: the counts are the whole
+ *    workspace; nothing until is_last, then both axes in two launches in place
+ *    on d_G;
+ *  - otherwise (smaller powers of two, sides above 1024, the other precisions):
+ *    the DFT along x of every scan row completed by this chunk, complex64
+ *    [scan_nx/2+1][scan_ny][P_pad]; with is_last the DFT along y.
  * Chunks must arrive in frame order starting at frame 0 (else EORDER).  With
  * is_last (the chunk ends at the last frame) d_G receives
  * G(k, K) = F_{R->K} counts: complex64 [scan_nx/2+1][P_pad][scan_ny]
