@@ -26,8 +26,7 @@
 // transformed.  (Seven kernels over the whole padded grid took 52 us a step on
 // 1024 x 1024, and 39 us with overlapping launches; these take 27 us.)  They
 // are bound by latency: 128 and 256 blocks, 15 MB in L2 (spectrum 8.4, fields 4.2,
-// COM maps 2.1).  Other grids take the
-// kernels over the whole grid below.
+// COM maps 2.1).  Other grids take the kernels over the whole grid below.
 #include "common.cuh"
 #include "fft_warp.cuh"
 

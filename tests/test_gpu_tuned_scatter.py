@@ -1,7 +1,7 @@
 """The autotuner's largest scatter shape is the built-in one: its timed range
 ends at three blocks per SM, where the kernel may fit more.  Launches of the
-two are timed in turn, the shortest of 20 each: the same launch, so within 3 %
-(three blocks instead of four took 5 % longer).
+two are timed in turn, the shortest of 20 each: the same launch, so within 5 %
+(three blocks instead of four took 12 % longer on these events).
 """
 
 import pytest
@@ -36,5 +36,5 @@ def test_three_blocks_mean_all_that_fit():
             rec.accumulate(idx, off)
             torch.cuda.synchronize()
             best[cps] = min(best[cps], ev[0][at].elapsed_time(ev[1][at]))
-    assert best[3] <= 1.03 * best[0], best
+    assert best[3] <= 1.05 * best[0], best
     assert rec.check() == 0
